@@ -52,7 +52,10 @@ extern "C" {
 #define BS_ERR_CUDA 4    /* a CUDA runtime call failed                          */
 #define BS_ERR_TIMEOUT 5 /* a bounded device-side wait gave up                  */
 
-#define BS_FP64 0 /* every step in float64                                           */
+#define BS_FP64 0 /* float64: every value and every sum keeps 53 bits or more (the    */
+                  /* far rule's as three float32 words each); a float32 test decides  */
+                  /* near or far, or a line's next face, only where its error bound   */
+                  /* leaves no doubt, else float64 does                               */
 #define BS_FP32 1 /* float32 bulk with compensated per-point sums; the ray steps of   */
                   /* pairs whose point sits on a vertex, edge or face of the tet run  */
                   /* in float64; the final per-point sum is float64                   */

@@ -21,8 +21,8 @@ constexpr double kPi = 3.14159265358979323846;
 // Far record (one per tet, rebuilt when the far rule changes): everything the
 // far rule and the near/far test need, streamed through shared memory, with
 // w'_q = -(w_q |V| / 4pi) omega(x_q) (sign and 1/4pi of Eq. 1 folded in).
-//   double: [c (3), rho^2] then per quadrature point [x_q', w'_q, B_q] as nine two-float values and a pad, in the tile
-//           frame and the tile's units (4 + 10 Q doubles; see far_records64_kernel)
+//   double: [c (3), rho^2] then per quadrature point [x_q', w'_q, B_q] as nine three-float values, in the tile frame and
+//           the tile's units (4 + 12 Q doubles; see far_records64_kernel)
 //   float : tile frame (coordinates relative to the tile origin o), in one of two layouts:
 //           quadrature-pair layout: [c - o (3), rho^2] then the quadrature points in pairs (a, b),
 //           five float4 per pair, every value stored as the pair (value_a, value_b) so that one
@@ -50,7 +50,7 @@ constexpr int kFarPointPairs = 1;
 template <typename T>
 __host__ __device__ constexpr int far_stride(int Q, int layout = kFarQuadPairs)
 {
-    return sizeof(T) == 4 ? (layout == kFarPointPairs ? 4 + 20 * Q : 4 + 20 * ((Q + 1) / 2)) : (4 + 10 * Q);
+    return sizeof(T) == 4 ? (layout == kFarPointPairs ? 4 + 20 * Q : 4 + 20 * ((Q + 1) / 2)) : (4 + 12 * Q);
 }
 constexpr int kNearF32Vec4 = 15;  // float4 per near record
 namespace nf32 {

@@ -252,8 +252,9 @@ __global__ void far_records32_kernel(const double *__restrict__ near64, const do
 }
 
 // float64 far record: [c (3), rho^2] as doubles, then per quadrature point the nine values [x_q', w'_q, B_q] as
-// two-float values (and a pad), in the tile's units: lengths times 2^-k, weights times 2^-kw, with k and kw such that
-// the tile's largest coordinate (or circumradius) and weight come to at most 1, so that no part leaves the float range.
+// three-float values, 24 words: the two leading words of each in turn, and the nine third words as bfloat16 (two to a
+// word, a pad of three halves); in the tile's units: lengths times 2^-k, weights times 2^-kw, with k and kw such that
+// the tile's largest coordinate (or circumradius) and weight come to less than 1, so that no part leaves the float range.
 // k and kw go to the tile's header (second float4, y and z, as integers), and w != 0 there marks a tile with a value
 // that is not finite.
 constexpr int kRec64Threads = 128;  // a multiple of every tile
@@ -288,7 +289,8 @@ __global__ void __launch_bounds__(kRec64Threads)
     if (!in) return;
     const double len = __longlong_as_double((long long)big[0][slot]), wt = __longlong_as_double((long long)big[1][slot]);
     const bool odd = !(len < (double)INFINITY) || !(len > 0.0) || !(wt < (double)INFINITY);
-    const int k = odd ? 0 : max(ilogb(len) + 1, -1000), kw = odd || wt == 0.0 ? 0 : max(ilogb(wt) + 1, -1000);
+    const int k = odd ? 0 : min(max(ilogb(len) + 1, -1000), 1000);
+    const int kw = odd || wt == 0.0 ? 0 : min(max(ilogb(wt) + 1, -1000), 1000);
     if (threadIdx.x % tile == 0) {
         float4 *g = hdr + 2 * (te / tile) + 1;
         *g = make_float4(g->x, __int_as_float(k), __int_as_float(kw), odd ? 1.f : 0.f);
@@ -306,9 +308,17 @@ __global__ void __launch_bounds__(kRec64Threads)
         xl = scale(xl, sl);
         wv = scale(wv, sw);
         const D3 B = cross(xl, wv);
-        float2 *g = reinterpret_cast<float2 *>(d + 4 + 10 * q);
-        const double vals[10] = {xl.x, xl.y, xl.z, wv.x, wv.y, wv.z, B.x, B.y, B.z, 0.0};
-        for (int j = 0; j < 10; ++j) g[j] = df_split(vals[j]);
+        float *g = reinterpret_cast<float *>(d + 4 + 12 * q);
+        const double vals[9] = {xl.x, xl.y, xl.z, wv.x, wv.y, wv.z, B.x, B.y, B.z};
+        unsigned third[10] = {};
+        for (int j = 0; j < 9; ++j) {
+            const tfl v = j < 3 && !odd ? tf_coordinate(vals[j]) : tf_split(vals[j]);
+            g[2 * j] = v.h;
+            g[2 * j + 1] = v.l;
+            third[j] = bf16_bits(v.t);
+        }
+        for (int j = 0; j < 5; ++j) g[18 + j] = __int_as_float((int)(third[2 * j] | third[2 * j + 1] << 16));
+        g[23] = 0.f;
     }
 }
 

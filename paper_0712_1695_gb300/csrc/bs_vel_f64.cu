@@ -1,4 +1,5 @@
-// bs_vel_f64.cu -- float64 instances of the velocity kernel (every rule; bound by the float64 pipe).
+// bs_vel_f64.cu -- float64 instances of the velocity kernel (every rule; bound by the float32 pipe, see the far sweep's three-float
+// values in bs_velocity_kernel.cuh).
 #include "bs_velocity_kernel.cuh"
 
 namespace bs {
