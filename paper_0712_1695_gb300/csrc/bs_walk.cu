@@ -825,9 +825,22 @@ __device__ __forceinline__ void walk_rec(WalkRec<double> &c, const double *__res
 }
 
 // The start of a float64 half-line from the float32 margins of walk_start_f32: the tet whose margin is clearly positive
-// holds the direction, and where every margin is clearly negative the half-line leaves the mesh at x; in between, the
-// margins are taken again in float64.
+// holds the direction, and where every margin is clearly negative the half-line leaves the mesh at x; in between, and
+// for a node whose faces are not staged, the margins are taken again in float64.  The staged gradients are the float64
+// record's, rounded (face_through_rounded): each component is good to 6e-8 of itself whatever the tet's shape, and a
+// margin to 3e-7.  From the float32 walk record g_0 = -(g_1 + g_2 + g_3) cancels in flat tets to 1e-7 of the largest
+// gradient, and 1 to 84 of 187000 half-lines of a mesh flattened 1e4 to 1e5 times started in a wrong tet or were dropped.
 constexpr float kStartClear = 1e-5f;
+__device__ __forceinline__ float4 face_through_rounded(const double *__restrict__ r, int k, int j)
+{
+    const int i = j + (j >= k ? 1 : 0);
+    double g[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        g[a] = i > 0 ? r[nf64::G + 3 * i - 3 + a] : -(r[nf64::G + a] + r[nf64::G + 3 + a] + r[nf64::G + 6 + a]);
+    const V3<float> f = mk((float)g[0], (float)g[1], (float)g[2]);
+    return make_float4(f.x, f.y, f.z, rsqrtf(dot3(f, f)));
+}
 __device__ __forceinline__ int walk_start_code(WalkStart st)
 {
     return st.T < 0 || st.best < -kStartTolF ? -1 : (st.T << 2 | st.k);
@@ -989,10 +1002,16 @@ __global__ void __launch_bounds__(kWalkThreads, sizeof(T) == 4 ? 8 : 4) walk_lin
         __syncwarp();
         for (int i = lane; i < n_staged; i += 32) {
             const int code = a.inc[e0 + i];
-            const float4 *r = a.wrec + (int64_t)(code >> 2) * kWalkRecVec4;
-            const float4 q0 = __ldg(r), q1 = __ldg(r + 1), q2 = __ldg(r + 2);
+            if constexpr (F) {
+                const float4 *r = a.wrec + (int64_t)(code >> 2) * kWalkRecVec4;
+                const float4 q0 = __ldg(r), q1 = __ldg(r + 1), q2 = __ldg(r + 2);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) slots[3 * i + j] = face_through(q0, q1, q2, code & 3, j);
+                for (int j = 0; j < 3; ++j) slots[3 * i + j] = face_through(q0, q1, q2, code & 3, j);
+            } else {
+                const double *r = a.near64 + (int64_t)(code >> 2) * kNearF64;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) slots[3 * i + j] = face_through_rounded(r, code & 3, j);
+            }
             s_code[wq][i] = code;
         }
         __syncwarp();
@@ -1000,10 +1019,11 @@ __global__ void __launch_bounds__(kWalkThreads, sizeof(T) == 4 ? 8 : 4) walk_lin
         for (int l = lb + lane; l < min(a.L, lb + kWalkLines); l += 32, n_tasks += 2) {
             const float4 ln = __ldg(a.lines32 + l);
             WalkStart sp, sm;
-            walk_start_f32(a, node, slots, s_code[wq], n_staged, mk(ln.x, ln.y, ln.z), sp, sm);
+            if (F || n_staged >= 0)
+                walk_start_f32(a, node, slots, s_code[wq], n_staged, mk(ln.x, ln.y, ln.z), sp, sm);
             int cp = walk_start_code(sp), cm = walk_start_code(sm);
             if constexpr (!F) {
-                if (!(fabsf(sp.best) > kStartClear) || !(fabsf(sm.best) > kStartClear)) {
+                if (n_staged < 0 || !(fabsf(sp.best) > kStartClear) || !(fabsf(sm.best) > kStartClear)) {
                     const dbl4 l64 = a.lines64[l];
                     WalkStart64 dp, dm;
                     walk_start_f64(a, node, nullptr, nullptr, -1, mk(l64.x, l64.y, l64.z), dp, dm);
