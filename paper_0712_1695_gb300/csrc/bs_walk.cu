@@ -851,13 +851,14 @@ __device__ __forceinline__ int walk_start_code(WalkStart64 st)
 }
 
 // The float64 walk's faces in float32, from the float32 walk record: the entry and exit faces and the next tet, when the
-// float32 values leave no doubt about them (clear).  With G the sum of the gradients' components and D that of x - v0,
-// a_i is good to 4e-7 (1 + G D) and b_i to 4e-7 G, so a parameter t_i = -a_i / b_i to a fifth of
-// e_i = 2e-6 (1 + G D + |t_i| G) / |b_i|; no doubt: no |b_i| within 1e-5 G of zero, the nearest face ahead nearer than
-// every other by the sum of their e_i, and so the last face behind, except at the node itself (there the faces through
-// it tie at t = 0).
+// float32 values leave no doubt about them (clear).  With G the sum of the gradients' components, X that of x's and D
+// that of x - v0's plus 2e-8 X (x and v0 are two words each here, their third are dropped: 2^-48 (X + V), which far from
+// the origin, from 5e7 edges on, outgrows the rest), a_i is good to 4e-7 (1 + G D) and b_i to 4e-7 G, so a parameter
+// t_i = -a_i / b_i to a fifth of e_i = 2e-6 (1 + G D + |t_i| G) / |b_i|; no doubt: no |b_i| within 1e-5 G of zero, the
+// nearest face ahead nearer than every other by the sum of their e_i, and so the last face behind, except at the node
+// itself (there the faces through it tie at t = 0).
 struct FloatCut {
-    float lo;
+    float lo;  // a lower bound: e_i below the parameter of the last face behind
     int fin, fout, next;
     bool clear;
 };
@@ -876,7 +877,8 @@ __device__ __forceinline__ FloatCut float_cut(const float4 *__restrict__ rg, con
     float G = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) G += fabsf(g[i].x) + fabsf(g[i].y) + fabsf(g[i].z);
-    const float D = 1.f + G * (kk < 0 ? fabsf(d0.x) + fabsf(d0.y) + fabsf(d0.z) : 0.f);
+    const float X = fabsf(xs[0]) + fabsf(xs[1]) + fabsf(xs[2]);
+    const float D = 1.f + G * (kk < 0 ? fabsf(d0.x) + fabsf(d0.y) + fabsf(d0.z) + 2e-8f * X : 0.f);
     float av[4], t[4], e[4];
     av[1] = dot3(g[1], d0);
     av[2] = dot3(g[2], d0);
@@ -910,6 +912,7 @@ __device__ __forceinline__ FloatCut float_cut(const float4 *__restrict__ rg, con
         if (ahead[i]) r.clear = r.clear && (i == r.fout || t[i] - hi > e[i] + eo);
         else r.clear = r.clear && (kk >= 0 || i == r.fin || r.lo - t[i] > e[i] + ei);
     }
+    r.lo -= ei;
     r.next = r.fout == 0 ? c.nb.x : r.fout == 1 ? c.nb.y : r.fout == 2 ? c.nb.z : c.nb.w;
     return r;
 }
