@@ -31,6 +31,7 @@ int fail(int code, const std::string &msg)
 
 int cuda_fail(cudaError_t e, const char *where)
 {
+    (void)cudaGetLastError();  // reported here: the next call's launch checks must not meet it again
     return fail(BS_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 

@@ -1,0 +1,89 @@
+"""Calls that meet the end of the memory they may allocate: the library's stream-ordered allocations come from the device's
+current memory pool, and a child process puts a pool of limited size there.
+
+A call that is refused for want of memory leaves the handle and the library as they were: the next one that fits gives the
+same numbers.
+"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+PRELUDE = '''
+import ctypes, sys
+sys.path.insert(0, %r)
+import numpy as np, torch
+import paper_0712_1695_gb300 as bs
+from paper_0712_1695_gb300.binding import BS_ERR_CUDA, BSError
+from workloads import config2_ring
+torch.cuda.init()
+torch.empty(1, device="cuda")
+cu = ctypes.CDLL("libcuda.so.1")
+
+
+class Props(ctypes.Structure):  # CUmemPoolProps: pinned device memory, no handles exported
+    _fields_ = [("type", ctypes.c_int), ("handles", ctypes.c_int), ("loc", ctypes.c_int), ("dev", ctypes.c_int),
+                ("sec", ctypes.c_void_p), ("max_size", ctypes.c_size_t), ("usage", ctypes.c_ushort),
+                ("reserved", ctypes.c_ubyte * 54)]
+
+
+def check(r):
+    assert r == 0, r
+
+
+def limit(mib):
+    torch.cuda.synchronize()
+    p = ctypes.c_void_p()
+    check(cu.cuMemPoolCreate(ctypes.byref(p), ctypes.byref(Props(1, 0, 1, 0, None, mib << 20, 0))))
+    check(cu.cuDeviceSetMemPool(0, p))
+
+
+m = config2_ring(24)  # 13824 nodes, 73002 tets
+x = torch.from_numpy(m.nodes).cuda()
+few = x[::50].contiguous()
+new = lambda: bs.Mesh(m.nodes, m.tets, m.omega)
+
+
+def call(h, pts, **p):
+    """The velocities, or None when there was no memory for the call."""
+    try:
+        v = h.bs_velocity(pts, **p).cpu().numpy()
+    except BSError as e:
+        assert e.code == BS_ERR_CUDA, e
+        return None
+    h.bs_status()
+    return v
+
+
+def close(a, b, tol):
+    return np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
+'''
+
+SCRIPTS = {
+    # the error of a refused call is not met again by the next one
+    "after a refused call": '''
+RAY = dict(far_ratio=2.0, tet_gauss_order=64, n_theta=4, n_phi=8, precision=bs.BS_FP32)
+limit(1024)
+want = call(new(), few, **RAY)
+limit(64)
+assert call(new(), few, **RAY) is None  # 183 MiB of far records
+limit(1024)
+got = call(new(), few, **RAY)
+assert np.array_equal(got, want)
+''',
+}
+
+
+@pytest.mark.parametrize("name", list(SCRIPTS))
+def test_limited_pool(name):
+    r = subprocess.run([sys.executable, "-c", PRELUDE % ROOT + SCRIPTS[name]], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
