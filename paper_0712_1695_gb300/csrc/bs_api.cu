@@ -259,6 +259,7 @@ cudaError_t ensure_far(bs_ctx *h, int prec, int Q, int tile, int layout, cudaStr
 {
     bs_ctx::FarTables &f = h->ft[prec];
     if (f.far && f.Q == Q && f.tile == tile && f.layout == layout && f.version == h->version) return cudaSuccess;
+    f.version = 0;  // until the last of them is built: a call refused in between must not leave the former ones' key
     cudaError_t e;
     if (h->rule.order != Q) {
         if (h->rule.bary) cudaFreeAsync(h->rule.bary, st);

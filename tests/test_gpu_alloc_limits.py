@@ -47,6 +47,24 @@ def limit(mib):
     check(cu.cuDeviceSetMemPool(0, p))
 
 
+def fill():
+    """Take what is left of the pool, down to pieces of 512 bytes."""
+    held = []
+    size = 1 << 30
+    while size >= 512:
+        q = ctypes.c_uint64()
+        if cu.cuMemAllocAsync(ctypes.byref(q), ctypes.c_size_t(size), None) == 0:
+            held.append(q)
+        else:
+            size >>= 1
+    return held
+
+
+def free(held):
+    for q in held:
+        check(cu.cuMemFreeAsync(q, None))
+
+
 m = config2_ring(24)  # 13824 nodes, 73002 tets
 x = torch.from_numpy(m.nodes).cuda()
 few = x[::50].contiguous()
@@ -62,10 +80,6 @@ def call(h, pts, **p):
         return None
     h.bs_status()
     return v
-
-
-def close(a, b, tol):
-    return np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
 '''
 
 SCRIPTS = {
@@ -79,6 +93,24 @@ assert call(new(), few, **RAY) is None  # 183 MiB of far records
 limit(1024)
 got = call(new(), few, **RAY)
 assert np.array_equal(got, want)
+''',
+    # tables half replaced by a call that was refused are not taken for the former ones
+    "refused between two calls": '''
+RAY = dict(far_ratio=2.0, tet_gauss_order=4, n_theta=4, n_phi=8, precision=bs.BS_FP64)
+tile = [bs.bs_variant_shape(bs.BS_FP64, 4, 0, v)["tile"] for v in range(bs.bs_num_variants(bs.BS_FP64, 4, 0))]
+big, small = tile.index(32), tile.index(16)
+limit(256)
+h = new()
+h.bs_set_variant(bs.BS_FP64, 4, 0, big)
+first = call(h, few, **RAY)
+h.bs_set_variant(bs.BS_FP64, 4, 0, small)
+held = fill()
+assert call(h, few, **RAY) is None  # twice the tile headers
+h.bs_set_variant(bs.BS_FP64, 4, 0, big)
+call(h, few, **RAY)
+free(held)
+again = call(h, few, **RAY)
+assert np.array_equal(again, first)
 ''',
 }
 
