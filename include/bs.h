@@ -64,9 +64,14 @@ extern "C" {
 #define BS_NEAR_EXACT 1 /* near tets by the exact integral of Eq. 1 over the tet (the       */
                         /* analytic near-field evaluation Section 1 compares against:       */
                         /* face and edge integrals in closed form, 6 logarithms and 12      */
-                        /* atan2 per tet) with float64 geometry; the logarithms and arc     */
-                        /* tangents in float64 (BS_FP64) or float32 (BS_FP32); no ray hits   */
-                        /* are counted                                                      */
+                        /* atan2 per tet); geometry, logarithms and arc tangents in float64 */
+                        /* (BS_FP64), or the geometry as two float32 words (48 bits) and    */
+                        /* the logarithms and arc tangents in float32 (BS_FP32); no ray     */
+                        /* hits are counted.  A handle keeps a table of 976 bytes per tet    */
+                        /* for each precision it was used with; one that finds no memory    */
+                        /* for it, or needs the memory for a call's other buffers, forms     */
+                        /* every pair from the mesh instead from then on, about four times   */
+                        /* as slowly                                                        */
 
 typedef struct bs_ctx *bs_handle;
 typedef struct bs_batch_ctx *bs_batch;

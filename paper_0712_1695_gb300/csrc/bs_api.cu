@@ -90,8 +90,10 @@ struct bs_ctx {
         size_t far_cap = 0, hdr_cap = 0, cls_cap = 0;  // allocated bytes
     };
     FarTables ft[2];  // [BS_FP64], [BS_FP32]
-    // the exact near rule's table per precision, for the mesh version it was built for
+    // the exact near rule's table per precision, for the mesh version it was built for (null: every pair from the
+    // near records, as in a handle that found no memory for the table)
     void *exact[2] = {nullptr, nullptr};
+    bool exact_refused = false;
     uint64_t exact_version[2] = {0, 0};
     // spatial order of the evaluation points
     int *perm = nullptr;
@@ -297,15 +299,30 @@ cudaError_t ensure_far(bs_ctx *h, int prec, int Q, int tile, int layout, cudaStr
     return cudaSuccess;
 }
 
+// The exact near rule's table, the last buffer of a call to be allocated: the rule can do without it, so a handle that
+// finds no memory for it keeps to the near records from then on (the same rule, four times as slow).  A stream capture
+// allocates none, and a table that it rebuilds counts as not built for the calls outside.
 cudaError_t ensure_exact(bs_ctx *h, int prec, cudaStream_t st)
 {
     if (h->n_tets == 0 || (h->exact[prec] && h->exact_version[prec] == h->version)) return cudaSuccess;
-    cudaError_t e;
-    if (!h->exact[prec] && (e = cudaMallocAsync(&h->exact[prec], 8 * (size_t)kExactTable * h->n_tets, st)) != cudaSuccess)
-        return e;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    if (!h->exact[prec]) {
+        if (h->exact_refused || cap != cudaStreamCaptureStatusNone) return cudaSuccess;
+        e = cudaMallocAsync(&h->exact[prec], 8 * (size_t)kExactTable * h->n_tets, st);
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            h->exact[prec] = nullptr;
+            h->exact_refused = true;
+            return cudaSuccess;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    h->exact_version[prec] = 0;
     if ((e = build_exact_table(h->near64, h->n_tets, prec, h->exact[prec], st)) != cudaSuccess) return e;
     if (h->prof) h->prof_all += 1;
-    h->exact_version[prec] = h->version;
+    if (cap == cudaStreamCaptureStatusNone) h->exact_version[prec] = h->version;
     return cudaSuccess;
 }
 
@@ -382,6 +399,17 @@ cudaError_t ensure_order(bs_ctx *h, int64_t k, int bits, cudaStream_t st)
     return cudaSuccess;
 }
 
+cudaError_t ensure_near_out(bs_ctx *h, size_t elems, cudaStream_t st)
+{
+    if (elems <= h->near_cap) return cudaSuccess;
+    if (h->near_out) cudaFreeAsync(h->near_out, st);
+    h->near_out = nullptr;
+    h->near_cap = 0;
+    const cudaError_t e = cudaMallocAsync((void **)&h->near_out, sizeof(double) * elems, st);
+    if (e == cudaSuccess) h->near_cap = elems;
+    return e;
+}
+
 cudaError_t ensure_partial(bs_ctx *h, size_t bytes, cudaStream_t st)
 {
     if (bytes <= h->partial_cap) return cudaSuccess;
@@ -391,6 +419,35 @@ cudaError_t ensure_partial(bs_ctx *h, size_t bytes, cudaStream_t st)
     cudaError_t e = cudaMallocAsync((void **)&h->partial, bytes, st);
     if (e == cudaSuccess) h->partial_cap = bytes;
     return e;
+}
+
+// When a buffer that a call cannot do without does not fit: gives back the exact near rule's tables, and with them what
+// grows with the points and may lie between them in the pool.  True when there was a table (outside a capture).  The host
+// waits for st here, so that the pool can return the pieces and take a larger one.
+bool drop_exact(bs_ctx *h, cudaStream_t st)
+{
+    if (!h->exact[0] && !h->exact[1]) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    (void)cudaGetLastError();  // the allocation that failed
+    auto give = [&](auto *&buf) {
+        if (buf) cudaFreeAsync(buf, st);
+        buf = nullptr;
+    };
+    give(h->exact[0]);
+    give(h->exact[1]);
+    h->exact_refused = true;
+    give(h->perm);
+    give(h->keys);
+    give(h->cell_count);
+    give(h->partial);
+    give(h->near_out);
+    h->order_cap = h->partial_cap = h->near_cap = 0;
+    h->cell_bits = 0;
+    cudaMemPool_t pool = nullptr;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return false;
+    if (cudaDeviceGetMemPool(&pool, h->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+    return true;
 }
 
 }  // namespace
@@ -917,7 +974,6 @@ int velocity_impl(bs_handle h, const double *eval_pts_dev, int64_t k, const bs_p
     }
     const int Q = p->tet_gauss_order;
     const int L = p->n_phi * p->n_theta;
-    BS_CUDA(ensure_lines(h, p->n_phi, p->n_theta, st));
     // far_ratio = +inf: every pair takes the ray rule, in the all-ray kernel (one point per thread,
     // direction windows, the direction table in shared memory: up to kRayLinesSmemMax lines);
     // BS_ALLRAY_GENERIC=1 keeps such calls on the velocity kernel
@@ -926,9 +982,6 @@ int velocity_impl(bs_handle h, const double *eval_pts_dev, int64_t k, const bs_p
                      p->near_rule == BS_NEAR_RAY;
     const int variant = ray ? 0 : choose_variant(h, p, k, near_walk != nullptr);
     const LaunchShape shape = ray ? ray_shape() : shape_for(p->precision, Q, variant, p->near_rule);
-    if (!ray) BS_CUDA(ensure_far(h, p->precision, Q, shape.tile, shape.layout, st));
-    const bool exact = p->near_rule == BS_NEAR_EXACT;
-    if (exact) BS_CUDA(ensure_exact(h, p->precision, st));
     int occ_ray = 0;
     if (ray) {
         if (h->ray_occ[p->precision] == 0 || h->ray_occ_L[p->precision] != L) {
@@ -964,8 +1017,31 @@ int velocity_impl(bs_handle h, const double *eval_pts_dev, int64_t k, const bs_p
     }
 
     const int bits = order_grid_bits(k);
-    BS_CUDA(ensure_order(h, k, bits, st));
-    BS_CUDA(ensure_partial(h, sizeof(double) * 3 * (size_t)k * n_chunks, st));
+    // the near pass evaluates the near pairs a variant leaves out of the far sweep: without the walk, few points split the
+    // tiles among several CTAs per group of 32 points (each part at least one group of 32 tiles per warp), for about
+    // kNearPassBlocksPerSm CTAs per SM in all
+    const bool near_pass = !ray && shape.drain == 3;
+    const int64_t groups = (k + 31) / 32;
+    int64_t split = 1;
+    if (near_pass && !near_walk) {
+        const int64_t tile_groups = (h->n_tets + 32LL * shape.tile - 1) / (32LL * shape.tile);
+        const int64_t want = ((int64_t)kNearPassBlocksPerSm * h->n_sm + groups - 1) / groups;
+        split = std::max<int64_t>(1, std::min<int64_t>({want, tile_groups / kNearPassWarps, 16}));
+    }
+    // the tables and buffers the call cannot do without
+    auto allocate = [&]() -> cudaError_t {
+        cudaError_t e = ensure_lines(h, p->n_phi, p->n_theta, st);
+        if (e == cudaSuccess && !ray) e = ensure_far(h, p->precision, Q, shape.tile, shape.layout, st);
+        if (e == cudaSuccess) e = ensure_order(h, k, bits, st);
+        if (e == cudaSuccess) e = ensure_partial(h, sizeof(double) * 3 * (size_t)k * n_chunks, st);
+        if (e == cudaSuccess && near_pass) e = ensure_near_out(h, 3 * (size_t)k * (size_t)split, st);
+        return e;
+    };
+    cudaError_t ea = allocate();
+    if (ea == cudaErrorMemoryAllocation && drop_exact(h, st)) ea = allocate();
+    if (ea != cudaSuccess) return cuda_fail(ea, "velocity: tables and buffers");
+    const bool exact = p->near_rule == BS_NEAR_EXACT;
+    if (exact) BS_CUDA(ensure_exact(h, p->precision, st));
     BS_CUDA(spatial_order(eval_pts_dev, k, bits, h->box, h->keys, h->cell_count, h->perm, st));
 
     VelocityArgs a;
@@ -998,24 +1074,7 @@ int velocity_impl(bs_handle h, const double *eval_pts_dev, int64_t k, const bs_p
     if (a.n_items > INT32_MAX) return fail(BS_ERR_ARG, "too many work items for one launch (points x tet chunks)");
     a.wait_polls = h->copy_wait_polls;
     a.withhold_copies = h->withhold_copies;
-    if (!ray && shape.drain == 3) {  // the near pass evaluates the near pairs the far sweep leaves out
-        // without the walk, few points split the tiles among several CTAs per group of 32 points (each part at
-        // least one group of 32 tiles per warp), for about kNearPassBlocksPerSm CTAs per SM in all
-        const int64_t groups = (k + 31) / 32;
-        const int64_t tile_groups = (h->n_tets + 32LL * shape.tile - 1) / (32LL * shape.tile);
-        int64_t split = 1;
-        if (!near_walk) {
-            const int64_t want = ((int64_t)kNearPassBlocksPerSm * h->n_sm + groups - 1) / groups;
-            split = std::max<int64_t>(1, std::min<int64_t>({want, tile_groups / kNearPassWarps, 16}));
-        }
-        const size_t need = 3 * (size_t)k * (size_t)split;
-        if (need > h->near_cap) {
-            if (h->near_out) cudaFreeAsync(h->near_out, st);
-            h->near_out = nullptr;
-            h->near_cap = 0;
-            BS_CUDA(cudaMallocAsync((void **)&h->near_out, sizeof(double) * need, st));
-            h->near_cap = need;
-        }
+    if (near_pass) {
         a.near_out = h->near_out;
         a.tile = shape.tile;
         a.far_stride = p->precision == BS_FP32 ? far_stride<float>(Q, shape.layout) : far_stride<double>(Q);
@@ -1322,7 +1381,6 @@ int bs_batch_velocity(bs_batch b, const bs_params *p, double *const *outs, void 
         bs_ctx *h = b->meshes[i];
         const bs_ctx::FarTables &f = h->ft[prec], before = f;
         BS_CUDA(ensure_far(h, prec, Q, shape.tile, shape.layout, st));
-        if (nr == BS_NEAR_EXACT) BS_CUDA(ensure_exact(h, prec, st));
         changed = changed || before.version != f.version || before.Q != f.Q || before.tile != f.tile ||
                   before.layout != f.layout;
         if (b->order_version[i] != h->version) {
@@ -1369,7 +1427,6 @@ int bs_batch_velocity(bs_batch b, const bs_params *p, double *const *outs, void 
         m.far = h->ft[prec].far;
         m.near32 = h->near32;
         m.near64 = h->near64;
-        m.exact = nr == BS_NEAR_EXACT ? h->exact[prec] : nullptr;
         m.tile_hdr = h->ft[prec].hdr;
         m.pts = h->nodes;
         m.perm = b->perm + b->point_begin[i];
@@ -1397,6 +1454,11 @@ int bs_batch_velocity(bs_batch b, const bs_params *p, double *const *outs, void 
         BS_CUDA(cudaMallocAsync((void **)&b->near_out, sizeof(double) * 3 * std::max<int64_t>(b->n_points, 1), st));
         changed = true;
     }
+    if (nr == BS_NEAR_EXACT)  // after every buffer the batch needs
+        for (int i = 0; i < n; ++i) {
+            BS_CUDA(ensure_exact(b->meshes[i], prec, st));
+            md[i].exact = b->meshes[i]->exact[prec];
+        }
     // The near field of a variant that leaves it out: at the meshes' nodes, the mesh walk of each mesh (its tables
     // prepared here, outside any capture) where the mesh allows it; the near pass skips those meshes.
     const int L = p->n_phi * p->n_theta;

@@ -2,7 +2,8 @@
 current memory pool, and a child process puts a pool of limited size there.
 
 A call that is refused for want of memory leaves the handle and the library as they were: the next one that fits gives the
-same numbers.
+same numbers.  The exact near rule's table per tet is an optimisation: a call that finds no room for it evaluates pair by pair, and a
+table already held makes way for buffers that a later call cannot do without.
 """
 import os
 import subprocess
@@ -65,10 +66,11 @@ def free(held):
         check(cu.cuMemFreeAsync(q, None))
 
 
-m = config2_ring(24)  # 13824 nodes, 73002 tets
+m = config2_ring(24)  # 13824 nodes, 73002 tets: a table of 68 MiB
 x = torch.from_numpy(m.nodes).cuda()
 few = x[::50].contiguous()
 new = lambda: bs.Mesh(m.nodes, m.tets, m.omega)
+EXACT = dict(far_ratio=2.0, tet_gauss_order=4, n_theta=4, n_phi=8, near_rule=bs.BS_NEAR_EXACT)
 
 
 def call(h, pts, **p):
@@ -80,6 +82,10 @@ def call(h, pts, **p):
         return None
     h.bs_status()
     return v
+
+
+def close(a, b, tol):
+    return np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
 '''
 
 SCRIPTS = {
@@ -111,6 +117,43 @@ call(h, few, **RAY)
 free(held)
 again = call(h, few, **RAY)
 assert np.array_equal(again, first)
+''',
+    # the table does not fit, the rest does
+    "no room for the table": '''
+for prec, tol in ((bs.BS_FP32, 1e-6), (bs.BS_FP64, 1e-12)):
+    limit(1024)
+    want = call(new(), few, precision=prec, **EXACT)
+    limit(64)
+    h = new()
+    for _ in range(2):
+        got = call(h, few, precision=prec, **EXACT)
+        assert got is not None and close(got, want, tol)
+    limit(1024)
+    full = call(new(), x, precision=prec, **EXACT)
+    limit(192)
+    h = [new(), new()]
+    b = bs.Batch(h)
+    outs = [torch.empty_like(x), torch.empty_like(x)]
+    b.bs_batch_velocity(outs, precision=prec, **EXACT)
+    torch.cuda.synchronize()
+    for o in outs:
+        assert close(o.cpu().numpy(), full, tol)
+''',
+    # what a handle can do does not depend on the table it holds
+    "the table makes way": '''
+worked = 0
+for mib in range(96, 513, 32):
+    limit(mib)
+    alone = call(new(), x, precision=bs.BS_FP32, **EXACT)
+    limit(mib)
+    h = new()
+    call(h, few, precision=bs.BS_FP32, **EXACT)
+    after = call(h, x, precision=bs.BS_FP32, **EXACT)
+    assert (after is None) == (alone is None), (mib, after is None)
+    if after is not None:
+        assert close(after, alone, 1e-6)
+        worked += 1
+assert worked
 ''',
 }
 
