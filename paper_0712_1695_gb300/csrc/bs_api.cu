@@ -256,13 +256,18 @@ cudaError_t ensure_lines(bs_ctx *h, int n_phi, int n_theta, cudaStream_t st)
 }
 
 // The far records of tet rule Q for a precision, in the float32 layout and tile size of the variant a call uses (the
-// tile headers and the tile frames depend on the tile), rebuilt when the mesh changed.
+// tile headers and the tile frames depend on the tile), rebuilt when the mesh changed.  Inside a stream capture (of a call
+// in the precision that no call outside has used yet) the buffers are the handle's own, not the graph's, and tables that
+// it builds count as not built for the calls outside, which may come before the graph runs.
 cudaError_t ensure_far(bs_ctx *h, int prec, int Q, int tile, int layout, cudaStream_t st)
 {
     bs_ctx::FarTables &f = h->ft[prec];
     if (f.far && f.Q == Q && f.tile == tile && f.layout == layout && f.version == h->version) return cudaSuccess;
     f.version = 0;  // until the last of them is built: a call refused in between must not leave the former ones' key
-    cudaError_t e;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
     if (h->rule.order != Q) {
         if (h->rule.bary) cudaFreeAsync(h->rule.bary, st);
         if (h->rule.w) cudaFreeAsync(h->rule.w, st);
@@ -274,13 +279,22 @@ cudaError_t ensure_far(bs_ctx *h, int prec, int Q, int tile, int layout, cudaStr
         h->rule.order = Q;
     }
     const size_t n = (size_t)std::max<int64_t>(h->n_tets, 1);
-    auto grow = [&](void **buf, size_t &cap, size_t bytes) -> cudaError_t {
-        if (bytes <= cap && *buf) return cudaSuccess;
-        if (*buf) cudaFreeAsync(*buf, st);
-        *buf = nullptr;
-        cap = 0;
-        cudaError_t r = cudaMallocAsync(buf, bytes, st);
-        if (r == cudaSuccess) cap = bytes;
+    auto grow = [&](void **buf, size_t &size, size_t bytes) -> cudaError_t {
+        if (bytes <= size && *buf) return cudaSuccess;
+        cudaError_t r;
+        if (!*buf && capturing) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // an allocation now, not a node of the graph
+            if ((r = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return r;
+            r = cudaMalloc(buf, bytes);
+            const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+            if (r == cudaSuccess) r = back;
+        } else {
+            if (*buf) cudaFreeAsync(*buf, st);
+            *buf = nullptr;
+            size = 0;
+            r = cudaMallocAsync(buf, bytes, st);
+        }
+        if (r == cudaSuccess) size = bytes;
         return r;
     };
     const bool f32 = prec == BS_FP32;
@@ -295,7 +309,7 @@ cudaError_t ensure_far(bs_ctx *h, int prec, int Q, int tile, int layout, cudaStr
     f.Q = Q;
     f.tile = tile;
     f.layout = layout;
-    f.version = h->version;
+    f.version = capturing ? 0 : h->version;
     return cudaSuccess;
 }
 
