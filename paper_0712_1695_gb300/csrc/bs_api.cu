@@ -119,6 +119,7 @@ struct bs_ctx {
     double *rk = nullptr;
     double *rk_w = nullptr;
     int occ[2][2][65][kMaxVariants] = {};  // cached CTAs per SM by [near rule][precision][Q][variant]
+    int walk_occ[2] = {};                  // cached CTAs per SM of the unheld float32 walk by [with the derivative]
     int ray_occ[2] = {};                   // cached CTAs per SM of the all-ray kernel by [precision]
     int ray_occ_L[2] = {};                 // ... for this many directions
     int pinned[2][2][65];                  // bs_set_variant by [near rule][precision][Q], -1: automatic
@@ -841,6 +842,11 @@ int nodes_impl(bs_handle h, const bs_params *p, double *out_dev, const double *d
         w.counts = p->counts;
         w.ready = ready;
         return velocity_impl(h, h->nodes, h->n_nodes, p, out_dev, stream, nullptr, &w);
+    }
+    if (p->precision == BS_FP32) {
+        int &occ = h->walk_occ[dout ? 1 : 0];
+        if (occ == 0) occ = std::max(1, walk_ctas_per_sm(dout != nullptr));
+        w.wave = occ * h->n_sm;
     }
     if (ready) BS_CUDA(cudaStreamWaitEvent(st, ready, 0));
     cudaEvent_t e0 = nullptr, e1 = nullptr;

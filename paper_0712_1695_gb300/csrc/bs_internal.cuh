@@ -356,6 +356,7 @@ struct WalkArgs {
     double far_ratio2 = 0.0;
     const float *r_stop = nullptr;    // device: max over tets of far_ratio * circumradius + bounding radius
     cudaEvent_t ready = nullptr;      // the walk's tables (null: queued on the walk's stream)
+    int wave = 0;                     // float32, all lines: CTAs of the unheld instance that the GPU takes at once
 };
 constexpr int kWalkRecVec4 = 8;  // float4 per float32 walk record (one 128-byte line)
 // float32 walk records from the near records and the face neighbours (after every mesh update)
@@ -371,6 +372,7 @@ cudaError_t launch_walk_finalize(const WalkGrid *g, int *mode, cudaStream_t st);
 cudaError_t launch_convex_check(const double *nodes, const int32_t *tets, const int32_t *nbr, int64_t n_tets,
                                 const int32_t *bface, int64_t n_bface, const int32_t *bnode, int64_t n_bnode,
                                 float4 *bpos, int conforming, int *mode, float4 *wrec, cudaStream_t st);
+int walk_ctas_per_sm(bool derivative);
 cudaError_t launch_walk(int precision, const WalkArgs &a, cudaStream_t st, cudaEvent_t ev_start = nullptr,
                         cudaEvent_t ev_stop = nullptr);
 // *r_stop := (1 + 1e-4) max over tets of (far_ratio * circumradius + bounding radius about the centroid):

@@ -628,13 +628,15 @@ __device__ V3<double> walk_f64(const WalkArgs &a, WalkStart64 st, V3<double> x, 
 // NEAR: the near field of the hybrid rule (see WalkArgs::near_mode), else the all-ray rule.
 // The float32 instances for convex domains without the derivative are held to 64 registers (8 CTAs, 32 warps per
 // SM): the walk waits on its dependent gathers, and the extra warps hide more of that than the few spills cost
-// (256-mesh batch 223 -> 219 ms, all-ray 64^3 173 -> 164 ms).  The near instance for non-convex ones to 73 (7 CTAs:
-// 28 warps, so that a 16^3 mesh's 4096 nodes are one wave of them; 91 registers took 20 warps: four Heun steps at 16^3
-// 5.26 -> 4.97 ms, 20^3 in a ball 2.62 -> 2.39; 6 CTAs 5.25 and 2.57, 8 with spills 5.04 and 2.53).
+// (256-mesh batch 223 -> 219 ms, all-ray 64^3 173 -> 164 ms).  The near instance for non-convex ones to 73 (7 CTAs, 28
+// warps; of 91 registers, 20 warps), at every size: its half-lines are short and wait on their loads, and the more warps the
+// better (Heun steps, four at 16^3 5.07 -> 4.68 ms, 24^3 22.6 -> 22.0, 32^3 99.4 -> 97.9; two at 48^3 488.8 -> 487.1, 64^3
+// 2680.9 -> 2675.2, where the walks take 2%; at 16^3 6 CTAs 5.25 against 4.97, 8 with spills 5.04).
 // FULL: the float32 instances of all lines on non-convex domains, to 7 CTAs (of 92 registers, 5 CTAs: 20^3 in a ball
 // 1.94 -> 1.75 ms; 6 CTAs 1.89, 8 CTAs 1.83) and with the derivative to 5 (of 108, 4 CTAs: 20^3 2.10 -> 1.87 ms, 36^3
-// 18.3 -> 16.4; 6 CTAs 1.92 and 16.4), for meshes with more nodes than the CTAs of the unheld instance take at once;
-// with fewer, the registers serve better (12^3 in a ball with the derivative: 0.595 ms, 0.605 held).
+// 18.3 -> 16.4; 6 CTAs 1.92 and 16.4), for meshes with more nodes than the CTAs of the unheld instance take at once
+// (WalkArgs::wave, from the device's SMs and that instance's occupancy); with fewer, the registers serve better (12^3 in a
+// ball with the derivative: 0.595 ms, 0.605 held).
 template <typename T, bool GRAD, bool RE, bool NEAR, bool FULL = false>
 __global__ void __launch_bounds__(kWalkThreads, sizeof(T) == 8 ? 1 : NEAR ? (RE ? 7 : 8) : !FULL ? 1 : GRAD ? 5 : 7)
     walk_kernel(const WalkArgs a)
@@ -1692,6 +1694,16 @@ cudaError_t launch_near_reach(const double *rho2, const double *near64, int64_t 
     return cudaGetLastError();
 }
 
+// CTAs per SM of the float32 all-lines walk on non-convex domains that is not held to a register bound
+int walk_ctas_per_sm(bool derivative)
+{
+    int n = 0;
+    const cudaError_t e =
+        derivative ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<float, true, true, false>, kWalkThreads, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<float, false, true, false>, kWalkThreads, 0);
+    return e == cudaSuccess ? n : 0;
+}
+
 cudaError_t launch_walk(int precision, const WalkArgs &a, cudaStream_t st, cudaEvent_t ev_start, cudaEvent_t ev_stop)
 {
     cudaError_t e;
@@ -1703,8 +1715,7 @@ cudaError_t launch_walk(int precision, const WalkArgs &a, cudaStream_t st, cudaE
         re<<<(unsigned)blocks, kWalkThreads, 0, st>>>(a);
     };
     const bool f32 = precision == BS_FP32;
-    // more nodes than 152 SMs take at once at the unheld instance's CTAs (walk_kernel, FULL)
-    const bool full = blocks > 152 * (a.dout ? 4 : 5);
+    const bool full = blocks > a.wave;  // walk_kernel, FULL
     if (a.near_mode) {
         if (a.dout || !a.perm || !a.near_out || !a.r_stop || (f32 ? !a.cls : !a.far)) return cudaErrorInvalidValue;
         if (f32) pair(walk_kernel<float, false, false, true>, walk_kernel<float, false, true, true>);
