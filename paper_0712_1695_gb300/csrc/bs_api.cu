@@ -1125,9 +1125,12 @@ int velocity_impl(bs_handle h, const double *eval_pts_dev, int64_t k, const bs_p
                 WalkArgs w = *near_walk;
                 w.perm = h->perm;
                 w.near_out = a.near_out;
-                w.far = a.m.far;
-                w.cls = ft.cls;
-                w.far_stride = a.far_stride;
+                if (p->precision == BS_FP64) {
+                    w.far = a.m.far;
+                    w.far_stride = a.far_stride;
+                } else {
+                    w.cls = ft.cls;
+                }
                 w.far_ratio2_f = a.far_ratio2_f;
                 w.far_ratio2 = a.far_ratio2;
                 w.counts = p->counts;
@@ -1510,9 +1513,12 @@ int bs_batch_velocity(bs_batch b, const bs_params *p, double *const *outs, void 
             w.near_mode = 1;
             w.perm = md[i].perm;
             w.near_out = b->near_out + 3 * md[i].point_begin;
-            w.far = md[i].far;
-            w.cls = h->ft[prec].cls;
-            w.far_stride = prec == BS_FP32 ? far_stride<float>(Q, shape.layout) : far_stride<double>(Q);
+            if (prec == BS_FP64) {
+                w.far = md[i].far;
+                w.far_stride = far_stride<double>(Q);
+            } else {
+                w.cls = h->ft[prec].cls;
+            }
             w.far_ratio2_f = fr2f;
             w.far_ratio2 = fr2;
             w.r_stop = h->r_stop;
