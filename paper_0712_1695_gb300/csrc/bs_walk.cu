@@ -636,9 +636,10 @@ __device__ V3<double> walk_f64(const WalkArgs &a, WalkStart64 st, V3<double> x, 
 // 1.94 -> 1.75 ms; 6 CTAs 1.89, 8 CTAs 1.83) and with the derivative to 5 (of 108, 4 CTAs: 20^3 2.10 -> 1.87 ms, 36^3
 // 18.3 -> 16.4; 6 CTAs 1.92 and 16.4), for meshes with more nodes than the CTAs of the unheld instance take at once
 // (WalkArgs::wave, from the device's SMs and that instance's occupancy); with fewer, the registers serve better (12^3 in a
-// ball with the derivative: 0.595 ms, 0.605 held).
+// ball with the derivative: 0.595 ms, 0.605 held).  Likewise all lines on convex ones where walk_lines_kernel is the slower
+// (use_lines_kernel), to 8 CTAs.
 template <typename T, bool GRAD, bool RE, bool NEAR, bool FULL = false>
-__global__ void __launch_bounds__(kWalkThreads, sizeof(T) == 8 ? 1 : NEAR ? (RE ? 7 : 8) : !FULL ? 1 : GRAD ? 5 : 7)
+__global__ void __launch_bounds__(kWalkThreads, sizeof(T) == 8 ? 1 : NEAR ? (RE ? 7 : 8) : !FULL ? 1 : GRAD ? 5 : RE ? 7 : 8)
     walk_kernel(const WalkArgs a)
 {
     static_assert(sizeof(T) == 4 || GRAD, "walk_lines_kernel is float64's walk without the derivative");
@@ -1694,6 +1695,18 @@ cudaError_t launch_near_reach(const double *rho2, const double *near64, int64_t 
     return cudaGetLastError();
 }
 
+// Which of the float32 kernels of all lines on convex domains (the same bits): walk_lines_kernel fetches the lanes' records
+// together and lets lanes run ahead, which pays where many warps walk lines that spread (time against walk_kernel's, 128
+// lines: 16^3 0.89, 20^3 0.74, 40^3 0.65).  With fewer than 8 lines most lanes idle (16^3 to 64^3: 1 line 1.15 to 1.28, 6
+// lines 1.01 to 1.10, 8 lines 0.92 to 1.0).  With many lines a node's neighbouring lanes walk the same tets, whose loads
+// coalesce by themselves, and on a small mesh the end of each turn of 128 lines counts: from 3/4 n^2 lines of an n^3 mesh or so
+// (64 at least) it is the slower one or not much the faster (10^3: 0.94 at 80 lines, 1.12 at 256; 18^3: 0.87 at 224, 1.09 at
+// 256; 24^3: 0.95 at 512, 1.15 at 1024; 32^3: 0.84 at 768, 1.04 at 1024; 5^3, 1024 lines: 1.49).
+bool use_lines_kernel(const WalkArgs &a)
+{
+    return a.L >= 8 && (a.L <= 64 || a.L <= 0.75 * std::pow((double)a.n_nodes, 2.0 / 3.0));
+}
+
 // CTAs per SM of the float32 all-lines walk on non-convex domains that is not held to a register bound
 int walk_ctas_per_sm(bool derivative)
 {
@@ -1725,8 +1738,11 @@ cudaError_t launch_walk(int precision, const WalkArgs &a, cudaStream_t st, cudaE
         else if (f32) pair(walk_kernel<float, true, false, false>, walk_kernel<float, true, true, false>);
         else pair(walk_kernel<double, true, false, false>, walk_kernel<double, true, true, false>);
     } else {
-        if (f32 && full) pair(walk_lines_kernel<float, false, false>, walk_kernel<float, false, true, false, true>);
-        else if (f32) pair(walk_lines_kernel<float, false, false>, walk_kernel<float, false, true, false>);
+        const bool lines = use_lines_kernel(a);
+        if (f32 && full && lines) pair(walk_lines_kernel<float, false, false>, walk_kernel<float, false, true, false, true>);
+        else if (f32 && lines) pair(walk_lines_kernel<float, false, false>, walk_kernel<float, false, true, false>);
+        else if (f32 && full) pair(walk_kernel<float, false, false, false, true>, walk_kernel<float, false, true, false, true>);
+        else if (f32) pair(walk_kernel<float, false, false, false>, walk_kernel<float, false, true, false>);
         else pair(walk_lines_kernel<double, false, false>, walk_lines_kernel<double, true, false>);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
