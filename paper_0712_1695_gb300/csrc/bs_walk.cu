@@ -790,7 +790,7 @@ __device__ __forceinline__ float dot_along(V3<float> g, V3<float> d, bool minus)
 // float64: the float64 pipe (a 72nd of float32's rate) was busy 86% of the time, four divisions a step first among it.
 //   The faces are cut in float32 (float_cut), and the tets that count take two divisions (chord_f64); where float32
 //   leaves a doubt the step is made in float64 as a whole.  The starts likewise (kStartClear).  9^3 nodes, order 4:
-//   1.185 -> 0.83 ms a call; 18^3: 10.6 -> 8.8; all lines at 12^3: 3.64 -> 2.13; 15^3 in a ball 12.5 -> 11.5.
+//   0.35 ms off a call; 18^3: 1.8; all lines at 12^3: 3.64 -> 2.13; 15^3 in a ball 12.5 -> 11.5.
 constexpr int kWalkSlot = kWalkRecVec4 + 1;      // float4 per slot
 constexpr int kWalkLines = 128;                  // lines per turn of a warp
 constexpr int kWalkOpen = 4;  // lanes without a half-line before the next are opened (all lines: 28.0 ms with 1, 28.6 with 8)
