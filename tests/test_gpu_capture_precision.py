@@ -52,4 +52,7 @@ def test_captured_in_the_other_precision(first, second, nodes, near_rule):
         assert close(out.cpu().numpy())
     del g
     assert np.array_equal(call(h, second).cpu().numpy(), want)
+    larger = dict(p, tet_gauss_order=64, precision=second)  # buffers that the capture allocated give way to larger ones
+    assert np.array_equal(h.bs_velocity(pts, out_dev=out, **larger).cpu().numpy(),
+                          plain.bs_velocity(pts, **larger).cpu().numpy())
     h.bs_status()
